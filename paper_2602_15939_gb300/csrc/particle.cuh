@@ -1009,9 +1009,12 @@ __device__ inline void deposit_1axis(const JA& ja, int cidx, const T o[3], const
     const T xa1 = oa + pick3(d, a), xb1 = ob + pick3(d, b), xc1 = oc + pick3(d, c);
     const int sa = stride(a), sb = stride(b), sc = stride(c);
     // axis a: the window of the full deposit; the particle moves to the next
-    // node up or down, so one shape fills the lower and one the upper nodes
+    // node up or down, so one shape fills the lower and one the upper nodes.
+    // Up or down by the arithmetic of cross_mask, not by the sign of the move:
+    // the largest number below 1/2 plus 1/2 rounds to 1, so a particle at rest
+    // there is nearest node 0 by its start and node 1 by its end.
     const T na = ORD == 1 ? T(0) : (oa >= T(0.5) ? T(1) : T(0));
-    const bool up = xa1 > oa;
+    const bool up = t_floor<T>(ORD == 1 ? xa1 : xa1 + T(0.5)) > na;
     const int wba = (na != T(0) ? 1 : 0) - (up ? 0 : 1) - (ORD == 1 ? 0 : 1);
     T S0a[NW], DSa[NW], CSa[NW - 1];
     {
