@@ -405,7 +405,7 @@ def measure(w, args, device, stream, rank, world, headline):
         best, ms_v, taken = box.autotune(4 if headline or w.n_particles > 1e8 else 2)
         tune = {"chosen": best, "how": f"autotuned on {taken} untimed steps",
                 "particle_ms_per_variant": [None if v is None else round(v, 4) for v in ms_v]}
-    nt_, st_, jc_ = P.pic_kernel_variant_info(tune["chosen"])
+    nt_, st_, jc_ = P.pic_get_launch_shape(box.h)
     tune.update({"threads_per_cta": nt_, "stable_order": bool(st_), "current_copies": jc_})
     if not args.variant and not w.fp64 and w.ndim == 3:
         cands = (2, 3, 4, 6)

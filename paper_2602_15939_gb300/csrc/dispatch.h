@@ -7,9 +7,9 @@
 namespace pic {
 
 struct KernelSet {
-    const void* tile[7];  // one per TILE_VARIANTS entry
+    const void* tile[8];  // one per TILE_SHAPES entry; null: not built (it does not fit, or is not taken there)
     const void* loose;
-    const void* batch;    // batched launch, variant batch_tile_variant
+    const void* batch;    // batched launch, shape batch_tile_shape
 };
 
 KernelSet lookup_f32_g0(int ord, int push, int esc);

@@ -1486,17 +1486,17 @@ constexpr long long TMA_WAIT_LIMIT = 1ll << 24;
 // (pick_copy); the flush sums the copies.  Particle states and FP32 currents
 // are the same in all variants (exact integer sums).
 struct TileVariant { int nt, stable, jc; };
-constexpr int N_TILE_VARIANTS = 7;
-constexpr TileVariant TILE_VARIANTS[N_TILE_VARIANTS] = {{256, 0, 1}, {512, 0, 1}, {512, 1, 1}, {256, 1, 1},
-                                                        {256, 0, 2}, {256, 1, 2}, {512, 0, 4}};
+constexpr int N_TILE_VARIANTS = 7;  // those a caller can ask for by number
+// Then the library's own shape for 4^3 tiles and FP64: variant 7 with half of
+// its threads.  It is taken when the choice is the library's or the
+// autotuner's and reported as variant 7 (its four copies); a caller who asks
+// for variant 7 gets the 512 threads that the table states.
+constexpr int N_TILE_SHAPES = 8, HALF_SHAPE = 7;
+constexpr TileVariant TILE_SHAPES[N_TILE_SHAPES] = {{256, 0, 1}, {512, 0, 1}, {512, 1, 1}, {256, 1, 1},
+                                                    {256, 0, 2}, {256, 1, 2}, {512, 0, 4}, {256, 0, 4}};
+constexpr bool has_half_shape(bool fp64, int geom) { return fp64 ? geom != G3D : geom == G3D_S; }
 
-// The shape variant v has on a tile geometry: the four current copies come
-// with 256 threads on 4^3 tiles and in FP64 (figures below).
-constexpr TileVariant tile_variant(bool fp64, int geom, int v) {
-    return v == 6 && (fp64 || geom == G3D_S) ? TileVariant{256, 0, 4} : TILE_VARIANTS[v];
-}
-
-// Variant (index) used when the choice is left to the library (measured on
+// Shape (index) used when the choice is left to the library (measured on
 // GB300).  3D FP32, 8^3 tiles: 512 threads with four current boxes.  4^3
 // tiles: the same four boxes with 256 threads, two CTAs per SM, so that one
 // tile's staging, zeroing and flush overlap the other's particles (a small
@@ -1510,10 +1510,10 @@ constexpr TileVariant tile_variant(bool fp64, int geom, int v) {
 // (particle kernel, us: 40 x 36 x 32 on 4^3 tiles 2132 -> 1638 against 512
 // threads with one, 64^2 in 2D 246 -> 212; 64^3 on 8^3 tiles with one copy
 // 7764 -> 7114).
-constexpr int default_tile_variant(bool fp64, int geom) {
-    return fp64 ? (geom == G3D ? 0 : 6) : (plane_of(geom) == G3D ? 6 : 1);
+constexpr int default_tile_shape(bool fp64, int geom) {
+    return has_half_shape(fp64, geom) ? HALF_SHAPE : (fp64 ? 0 : (geom == G3D ? 6 : 1));
 }
-constexpr int batch_tile_variant(bool fp64, int geom) { return default_tile_variant(fp64, geom); }
+constexpr int batch_tile_shape(bool fp64, int geom) { return default_tile_shape(fp64, geom); }
 
 // CTAs per SM the register budget is set for
 constexpr int tile_ctas(int nt, int jc) { return jc >= 4 ? (nt == 256 ? 2 : 1) : (nt == 512 ? 2 : 3); }
@@ -1613,6 +1613,16 @@ template <class T, int G, int NT, int STABLE, int JC> struct SmemLayout {
     static constexpr size_t QOD = (size_t)(NT / 32) * QN * 6 * sizeof(T);
     static constexpr size_t bytes = off_q + QE * QN * (NT / 32);
 };
+
+// Shared memory of launch shape V; NO_SHAPE where it is not built.
+constexpr size_t NO_SHAPE = ~(size_t)0;
+template <class T, int G, int V> constexpr size_t shape_bytes() {
+    constexpr TileVariant tv = TILE_SHAPES[V];
+    if constexpr (V == HALF_SHAPE && !has_half_shape(sizeof(T) == 8, G))
+        return NO_SHAPE;
+    else
+        return SmemLayout<T, G, tv.nt, tv.stable, tv.jc>::bytes;
+}
 
 // The fused particle step for tile t of one box (see the file header), made
 // by a CTA of NT threads whose mbarrier is initialised; parity: the phase of

@@ -64,23 +64,19 @@ struct Prof {
 
 }  // namespace
 
-// Shared memory of the particle kernel of variant v (E and B boxes, the
-// variant's current copies, barrier and counters).
-template <class T, int G, int V> static size_t smem_v() {
-    constexpr TileVariant tv = tile_variant(sizeof(T) == 8, G, V);
-    return SmemLayout<T, G, tv.nt, tv.stable, tv.jc>::bytes;
-}
-
+// Shared memory of the particle kernel of shape v (E and B boxes, the shape's
+// current copies, barrier and counters).
 template <class T, int G> static size_t tile_smem_bytes_t(int v) {
-    static_assert(N_TILE_VARIANTS == 7, "one entry per tile variant");
+    static_assert(N_TILE_SHAPES == 8, "one entry per shape");
     switch (v) {
-        case 0: return smem_v<T, G, 0>();
-        case 1: return smem_v<T, G, 1>();
-        case 2: return smem_v<T, G, 2>();
-        case 3: return smem_v<T, G, 3>();
-        case 4: return smem_v<T, G, 4>();
-        case 6: return smem_v<T, G, 6>();
-        default: return smem_v<T, G, 5>();
+        case 0: return shape_bytes<T, G, 0>();
+        case 1: return shape_bytes<T, G, 1>();
+        case 2: return shape_bytes<T, G, 2>();
+        case 3: return shape_bytes<T, G, 3>();
+        case 4: return shape_bytes<T, G, 4>();
+        case 5: return shape_bytes<T, G, 5>();
+        case 6: return shape_bytes<T, G, 6>();
+        default: return shape_bytes<T, G, 7>();
     }
 }
 
@@ -108,15 +104,18 @@ static size_t tile_smem_bytes(bool fp64, int tg, int v) {
     }
 }
 
-// Variant used when the configuration leaves the choice to the library
+// Shape used when the configuration leaves the choice to the library
 // (pic_autotune refines it for a given box).  2D FP32 with quadratic shapes
 // takes 256 threads: twice the registers of the 512-thread shape, which the 27
 // adds of its deposit need (particle kernel, us: 160^2 expanding box on 8 x 8
 // tiles 41.5 -> 37.3, 200 x 136 leaky box 156 -> 130, 400^2 on 16 x 16 298 ->
 // 294; with linear shapes 512 threads are as fast or faster).
-static int default_variant(bool fp64, int tg, int order) {
-    return !fp64 && plane_of(tg) != G3D && order == 2 ? 0 : default_tile_variant(fp64, tg);
+static int default_shape(bool fp64, int tg, int order) {
+    return !fp64 && plane_of(tg) != G3D && order == 2 ? 0 : default_tile_shape(fp64, tg);
 }
+
+// The number a shape goes by in the interface.
+static int variant_number(int shape) { return shape == HALF_SHAPE ? 7 : shape + 1; }
 
 // Steps between regroups of the particles by cell (0: never).  FP64 boxes do
 // not regroup: the order of their current's floating-point adds would then
@@ -134,8 +133,8 @@ struct pic_handle {
     int push = PUSH_BORIS, esc = ESC_NONE;
     KernelSet ks{};
     const void* tile_fn = nullptr;
-    int tile_variant = 1;  // index into TILE_VARIANTS
-    bool variant_auto = true;  // the library's choice: follows the tile shape
+    int tile_shape = 1;  // index into TILE_SHAPES
+    bool variant_auto = true;  // the launch shape is the library's choice: follows the tiles
     int tile_threads = 512;
     size_t smem_bytes = 0;
     int sms = 152;
@@ -665,7 +664,7 @@ template <class T, int G> static pic_status regroup_attr_t(pic_handle* h) {
 // tiles fills the GPU as it is, and every further CTA stages the fields and
 // flushes the current again.
 static int species_split(const pic_handle* h, int nsp) {
-    const TileVariant v = tile_variant(h->fp64, h->tg, h->tile_variant);
+    const TileVariant v = TILE_SHAPES[h->tile_shape];
     const int per_sm = std::max(1, std::min(tile_ctas(v.nt, v.jc), (int)(MAX_SMEM / (h->smem_bytes + 1024))));
     return nsp > 1 && (long long)h->tl.ntiles * nsp <= (long long)h->sms * per_sm ? nsp : 1;
 }
@@ -1586,23 +1585,23 @@ pic_status pic_init(const pic_config* cfg, pic_handle** out) {
         h->sms = 152;
     }
     {
-        int v = c.kernel_variant > 0 ? (int)c.kernel_variant - 1 : default_variant(h->fp64, h->tg, c.shape_order);
+        int v = c.kernel_variant > 0 ? (int)c.kernel_variant - 1 : default_shape(h->fp64, h->tg, c.shape_order);
         h->variant_auto = c.kernel_variant == 0;
         if (c.kernel_variant == 0)
             if (const char* e = getenv("PIC_KERNEL_VARIANT")) {
                 v = atoi(e) - 1;
                 h->variant_auto = false;
             }
-        if (v < 0 || v >= N_TILE_VARIANTS || tile_smem_bytes(h->fp64, h->tg, v) > MAX_SMEM) {
+        if (v < 0 || v >= (h->variant_auto ? N_TILE_SHAPES : N_TILE_VARIANTS) || tile_smem_bytes(h->fp64, h->tg, v) > MAX_SMEM) {
             delete h;
             return fail(nullptr, PIC_ERR_ARG, "particle-kernel variant %d does not fit this configuration", v + 1);
         }
-        h->tile_variant = v;
-        h->tile_threads = tile_variant(h->fp64, h->tg, v).nt;
+        h->tile_shape = v;
+        h->tile_threads = TILE_SHAPES[v].nt;
         h->smem_bytes = tile_smem_bytes(h->fp64, h->tg, v);
     }
     h->ks = lookup_kernels(h->fp64, h->tg, c.shape_order, h->push, h->esc);
-    h->tile_fn = h->ks.tile[h->tile_variant];
+    h->tile_fn = h->ks.tile[h->tile_shape];
 
     auto bail = [&](pic_status s) {
         g_init_error = h->last_error;
@@ -2064,7 +2063,7 @@ pic_status pic_preload_kernels(int32_t device, int32_t precision) {
             for (const auto& pe : pushes) {
                 const KernelSet ks = lookup_kernels(fp64, tg, ord, pe[0], pe[1]);
                 for (const void* f : ks.tile)
-                    if (cudaFuncGetAttributes(&a, f) != cudaSuccess) return fail(nullptr, PIC_ERR_CUDA, "kernel load failed");
+                    if (f && cudaFuncGetAttributes(&a, f) != cudaSuccess) return fail(nullptr, PIC_ERR_CUDA, "kernel load failed");
                 if (cudaFuncGetAttributes(&a, ks.loose) != cudaSuccess || cudaFuncGetAttributes(&a, ks.batch) != cudaSuccess)
                     return fail(nullptr, PIC_ERR_CUDA, "kernel load failed");
             }
@@ -2077,34 +2076,47 @@ int pic_kernel_variant_count(void) { return N_TILE_VARIANTS; }
 
 pic_status pic_kernel_variant_info(int32_t k, int32_t* threads_per_cta, int32_t* stable, int32_t* copies) {
     if (k < 1 || k > N_TILE_VARIANTS) return fail(nullptr, PIC_ERR_ARG, "kernel variant %d out of range", (int)k);
-    if (threads_per_cta) *threads_per_cta = TILE_VARIANTS[k - 1].nt;
-    if (stable) *stable = TILE_VARIANTS[k - 1].stable;
-    if (copies) *copies = TILE_VARIANTS[k - 1].jc;
+    if (threads_per_cta) *threads_per_cta = TILE_SHAPES[k - 1].nt;
+    if (stable) *stable = TILE_SHAPES[k - 1].stable;
+    if (copies) *copies = TILE_SHAPES[k - 1].jc;
     return PIC_OK;
 }
 
 pic_status pic_get_kernel_variant(pic_handle* h, int32_t* k) {
     if (!h || !k) return fail(h, PIC_ERR_ARG, "NULL argument");
-    *k = h->tile_variant + 1;
+    *k = variant_number(h->tile_shape);
+    return PIC_OK;
+}
+
+pic_status pic_get_launch_shape(pic_handle* h, int32_t* threads_per_cta, int32_t* stable, int32_t* copies) {
+    if (!h) return fail(h, PIC_ERR_ARG, "handle is NULL");
+    if (threads_per_cta) *threads_per_cta = TILE_SHAPES[h->tile_shape].nt;
+    if (stable) *stable = TILE_SHAPES[h->tile_shape].stable;
+    if (copies) *copies = TILE_SHAPES[h->tile_shape].jc;
+    return PIC_OK;
+}
+
+// Switch to launch shape v (index into TILE_SHAPES), which fits.
+static pic_status set_shape(pic_handle* h, int v) {
+    const size_t smem = tile_smem_bytes(h->fp64, h->tg, v);
+    if (smem > MAX_SMEM)
+        return fail(h, PIC_ERR_ARG, "kernel variant %d needs %zu bytes of shared memory", variant_number(v), smem);
+    cudaSetDevice(h->cfg.device);
+    if (cudaFuncSetAttribute(h->ks.tile[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return fail(h, PIC_ERR_CUDA, "cannot set %zu bytes of dynamic shared memory", smem);
+    drop_graphs(h);
+    h->tile_shape = v;
+    h->variant_auto = false;
+    h->tile_threads = TILE_SHAPES[v].nt;
+    h->smem_bytes = smem;
+    h->tile_fn = h->ks.tile[v];
     return PIC_OK;
 }
 
 pic_status pic_set_kernel_variant(pic_handle* h, int32_t k) {
     if (!h) return fail(h, PIC_ERR_ARG, "handle is NULL");
     if (k < 1 || k > N_TILE_VARIANTS) return fail(h, PIC_ERR_ARG, "kernel variant %d out of range", (int)k);
-    const int v = k - 1;
-    const size_t smem = tile_smem_bytes(h->fp64, h->tg, v);
-    if (smem > MAX_SMEM) return fail(h, PIC_ERR_ARG, "kernel variant %d needs %zu bytes of shared memory", (int)k, smem);
-    cudaSetDevice(h->cfg.device);
-    if (cudaFuncSetAttribute(h->ks.tile[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return fail(h, PIC_ERR_CUDA, "cannot set %zu bytes of dynamic shared memory", smem);
-    drop_graphs(h);
-    h->tile_variant = v;
-    h->variant_auto = false;
-    h->tile_threads = tile_variant(h->fp64, h->tg, v).nt;
-    h->smem_bytes = smem;
-    h->tile_fn = h->ks.tile[v];
-    return PIC_OK;
+    return set_shape(h, k - 1);
 }
 
 pic_status pic_autotune_regroup(pic_handle* h, const int32_t* candidates, int32_t n, int32_t cycles, int32_t* best,
@@ -2167,11 +2179,12 @@ pic_status pic_autotune_regroup(pic_handle* h, const int32_t* candidates, int32_
 static pic_status switch_tiling(pic_handle* h, int tg) {
     h->tg = tg;
     set_tiling(h);
-    int v = h->tile_variant;
-    if (h->variant_auto || tile_smem_bytes(h->fp64, tg, v) > MAX_SMEM) v = default_variant(h->fp64, tg, h->cfg.shape_order);
+    int v = h->tile_shape;
+    if (v == HALF_SHAPE && !has_half_shape(h->fp64, tg)) v = 6;  // the tuned number on other tiles
+    if (h->variant_auto || tile_smem_bytes(h->fp64, tg, v) > MAX_SMEM) v = default_shape(h->fp64, tg, h->cfg.shape_order);
     h->ks = lookup_kernels(h->fp64, tg, h->cfg.shape_order, h->push, h->esc);
-    h->tile_variant = v;
-    h->tile_threads = tile_variant(h->fp64, tg, v).nt;
+    h->tile_shape = v;
+    h->tile_threads = TILE_SHAPES[v].nt;
     h->smem_bytes = tile_smem_bytes(h->fp64, tg, v);
     h->tile_fn = h->ks.tile[v];
     if (cudaFuncSetAttribute(h->tile_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem_bytes) != cudaSuccess)
@@ -2254,7 +2267,7 @@ static pic_status retile(pic_handle* h, int tg) {
         return PIC_OK;
     };
     const int old_tg = h->tg;
-    const int old_variant = h->tile_variant;
+    const int old_shape = h->tile_shape;
     drop_species();
     h->buf = 0;
     pic_status st = switch_tiling(h, tg);
@@ -2262,7 +2275,7 @@ static pic_status retile(pic_handle* h, int tg) {
     if (st != PIC_OK) {
         const std::string why = h->last_error;
         drop_species();
-        h->tile_variant = old_variant;
+        h->tile_shape = old_shape;
         pic_status back = switch_tiling(h, old_tg);
         if (back == PIC_OK) back = load_all();
         free_flat();
@@ -2299,11 +2312,11 @@ pic_status pic_autotune(pic_handle* h, int32_t trial_steps, int32_t* best, doubl
     if (trial_steps < 1) return fail(h, PIC_ERR_ARG, "trial_steps must be >= 1");
     cudaSetDevice(h->cfg.device);
     const bool prof_was = h->prof.on;
-    const int start_variant = h->tile_variant;
-    double ms[N_TILE_VARIANTS];
-    long long launches[N_TILE_VARIANTS];
-    bool fits[N_TILE_VARIANTS];
-    for (int v = 0; v < N_TILE_VARIANTS; ++v) {
+    const int start_shape = h->tile_shape;
+    double ms[N_TILE_SHAPES];
+    long long launches[N_TILE_SHAPES];
+    bool fits[N_TILE_SHAPES];
+    for (int v = 0; v < N_TILE_SHAPES; ++v) {
         ms[v] = 0.0;
         launches[v] = 0;
         fits[v] = tile_smem_bytes(h->fp64, h->tg, v) <= MAX_SMEM;
@@ -2318,9 +2331,9 @@ pic_status pic_autotune(pic_handle* h, int32_t trial_steps, int32_t* best, doubl
     const long long l0 = h->prof.launches, pl0 = h->prof.particle_launches, ps0 = h->prof.particle_steps;
     pic_status st = PIC_OK;
     for (int r = 0; r < rounds && st == PIC_OK; ++r)
-        for (int v = 0; v < N_TILE_VARIANTS && st == PIC_OK; ++v) {
+        for (int v = 0; v < N_TILE_SHAPES && st == PIC_OK; ++v) {
             if (!fits[v]) continue;
-            st = pic_set_kernel_variant(h, v + 1);
+            st = set_shape(h, v);
             if (st != PIC_OK) break;
             h->prof.on = false;
             st = pic_step(h, 1);  // first launch of the variant: not timed
@@ -2345,17 +2358,24 @@ pic_status pic_autotune(pic_handle* h, int32_t trial_steps, int32_t* best, doubl
     h->prof.particle_steps = ps0;
     h->prof.on = prof_was;
     if (st != PIC_OK) {
-        pic_set_kernel_variant(h, start_variant + 1);
+        set_shape(h, start_shape);
         return st;
     }
-    int bv = start_variant;
-    for (int v = 0; v < N_TILE_VARIANTS; ++v)
+    int bv = start_shape;
+    for (int v = 0; v < N_TILE_SHAPES; ++v)
         if (fits[v] && launches[v] > 0 && (launches[bv] == 0 || ms[v] / launches[v] < ms[bv] / launches[bv])) bv = v;
-    st = pic_set_kernel_variant(h, bv + 1);
+    st = set_shape(h, bv);
     if (st != PIC_OK) return st;
-    if (best) *best = bv + 1;
-    if (ms_per_variant)
-        for (int v = 0; v < N_TILE_VARIANTS; ++v) ms_per_variant[v] = launches[v] > 0 ? ms[v] / launches[v] : -1.0;
+    if (best) *best = variant_number(bv);
+    if (ms_per_variant) {
+        for (int k = 0; k < N_TILE_VARIANTS; ++k) ms_per_variant[k] = -1.0;
+        for (int v = 0; v < N_TILE_SHAPES; ++v) {
+            if (launches[v] <= 0) continue;
+            double& m = ms_per_variant[variant_number(v) - 1];  // the faster of a number's shapes
+            const double t = ms[v] / launches[v];
+            if (m < 0.0 || t < m) m = t;
+        }
+    }
     if (steps_taken) *steps_taken = taken;
     return PIC_OK;
 }
@@ -2378,16 +2398,15 @@ pic_status pic_autotune_tile(pic_handle* h, int32_t trial_steps, int32_t* best_s
     const double ms0[3] = {h->prof.ms[0], h->prof.ms[1], h->prof.ms[2]};
     const long long l0 = h->prof.launches, pl0 = h->prof.particle_launches, ps0 = h->prof.particle_steps;
     double per[3] = {-1.0, -1.0, -1.0};
-    int var[3] = {0, 0, 0};
+    int shape[3] = {-1, -1, -1};
     pic_status st = PIC_OK;
     for (int k = 0; k < nsides && st == PIC_OK; ++k) {
         st = pic_set_tile(h, sides[k]);
         if (st != PIC_OK) break;
         // the best launch variant for these tiles, then whole steps with it
-        int32_t bv = 0;
-        st = pic_autotune(h, trial_steps, &bv, nullptr, nullptr);
+        st = pic_autotune(h, trial_steps, nullptr, nullptr, nullptr);
         if (st != PIC_OK) break;
-        var[k] = bv;
+        shape[k] = h->tile_shape;
         h->prof.on = false;
         st = pic_step(h, 1);
         if (st != PIC_OK) break;
@@ -2414,7 +2433,7 @@ pic_status pic_autotune_tile(pic_handle* h, int32_t trial_steps, int32_t* best_s
     for (int k = 1; k < nsides; ++k)
         if (per[k] >= 0.0 && per[k] < per[b]) b = k;
     st = pic_set_tile(h, sides[b]);
-    if (st == PIC_OK && var[b] > 0) st = pic_set_kernel_variant(h, var[b]);
+    if (st == PIC_OK && shape[b] >= 0) st = set_shape(h, shape[b]);
     if (st != PIC_OK) return st;
     if (best_side) *best_side = sides[b];
     if (ms_per_side)
@@ -2840,8 +2859,8 @@ pic_status pic_batch_create(pic_handle* const* boxes, int32_t n, pic_batch** out
     B->fp64 = h0->fp64;
     B->tg = h0->tg;
     B->kern = h0->ks.batch;
-    const int v = batch_tile_variant(B->fp64, B->tg);
-    B->nt = tile_variant(B->fp64, B->tg, v).nt;
+    const int v = batch_tile_shape(B->fp64, B->tg);
+    B->nt = TILE_SHAPES[v].nt;
     B->smem = tile_smem_bytes(B->fp64, B->tg, v);
     int sms = 0, per_sm = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, B->device);

@@ -123,6 +123,7 @@ _SIGS = {
     "pic_kernel_variant_count": (C.c_int, []),
     "pic_kernel_variant_info": (C.c_int, [C.c_int32, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
     "pic_get_kernel_variant": (C.c_int, [_H, C.POINTER(C.c_int32)]),
+    "pic_get_launch_shape": (C.c_int, [_H, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
     "pic_set_kernel_variant": (C.c_int, [_H, C.c_int32]),
     "pic_take_result": (C.c_int, [_H, C.c_uint64, C.POINTER(_H)]),
     "pic_get_tile": (C.c_int, [_H, C.POINTER(C.c_int32)]),
@@ -359,6 +360,14 @@ def pic_get_kernel_variant(h) -> int:
     k = C.c_int32()
     _check(h, lib().pic_get_kernel_variant(h, C.byref(k)))
     return k.value
+
+
+def pic_get_launch_shape(h):
+    """(threads per CTA, stable stayer order 0/1, current-box copies) of the
+    particle kernel that h runs."""
+    nt, st, jc = C.c_int32(), C.c_int32(), C.c_int32()
+    _check(h, lib().pic_get_launch_shape(h, C.byref(nt), C.byref(st), C.byref(jc)))
+    return nt.value, st.value, jc.value
 
 
 def pic_set_kernel_variant(h, k: int):
