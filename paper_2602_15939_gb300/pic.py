@@ -146,6 +146,7 @@ _SIGS = {
     "pic_poll": (C.c_int, [C.c_void_p, C.c_uint64, C.POINTER(C.c_int), C.POINTER(pic_diag), C.POINTER(C.c_double)]),
     "pic_server_wait": (C.c_int, [C.c_void_p, C.c_uint64, C.c_double]),
     "pic_server_stats": (C.c_int, [C.c_void_p, C.POINTER(pic_server_info)]),
+    "pic_server_peak_concurrency": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32)]),
     "pic_server_destroy": (C.c_int, [C.c_void_p]),
     "pic_server_set_batching": (C.c_int, [C.c_void_p, C.c_int]),
 }
@@ -653,6 +654,12 @@ class Server:
         s = pic_server_info()
         _check(None, lib().pic_server_stats(self.h, C.byref(s)))
         return s
+
+    def peak_concurrency(self) -> int:
+        """The most runs that were running at once (pic_server_peak_concurrency)."""
+        n = C.c_int32()
+        _check(None, lib().pic_server_peak_concurrency(self.h, C.byref(n)))
+        return n.value
 
     def close(self):
         if self.h:
