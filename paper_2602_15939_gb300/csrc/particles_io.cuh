@@ -165,12 +165,14 @@ __global__ void __launch_bounds__(SCAN_THREADS) tile_offsets_kernel(int ntiles, 
 
 // Copy tile t's particles (front and back segments) to double arrays at
 // offset off[t]: absolute positions, momenta, ids, displacements.  limit: the
-// arrays' room.
+// arrays' room.  total (null: already checked on the host): the number of
+// particles; where it is not `limit` nothing is written.
 template <class T, int G>
 __global__ void compact_kernel(Tiling tl, Grid g, PView<T> v, const int* __restrict__ stay, const int* __restrict__ arr,
                                long long tcap, const long long* __restrict__ off, int t_first, long long o_first,
-                               long long limit, bool has_dr, double* __restrict__ x, double* __restrict__ u, uint32_t* __restrict__ id,
-                               double* __restrict__ dr) {
+                               long long limit, const long long* __restrict__ total, bool has_dr, double* __restrict__ x,
+                               double* __restrict__ u, uint32_t* __restrict__ id, double* __restrict__ dr) {
+    if (total && *total != limit) return;
     // tiles t_first + blockIdx.x; output index off[t] - o_first + i
     const int t = t_first + blockIdx.x;
     const int nst = stay[t], nar = arr[t];
@@ -200,8 +202,12 @@ template <class T, int G>
 __global__ void compact_loose_kernel(PView<T> v, const int* __restrict__ lcount, long long lcap, long long off0,
                                      const long long* __restrict__ off0_dev, long long limit, bool has_dr, double* __restrict__ x, double* __restrict__ u, uint32_t* __restrict__ id,
                                      double* __restrict__ dr) {
-    // at offset off0, or *off0_dev where that is given
-    if (off0_dev) off0 = *off0_dev;
+    // at offset off0, or off0_dev[0] where that is given, with the number of
+    // particles after it (compact_kernel)
+    if (off0_dev) {
+        if (off0_dev[1] != limit) return;
+        off0 = off0_dev[0];
+    }
     long long n = *lcount;
     if (n > lcap) n = lcap;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {

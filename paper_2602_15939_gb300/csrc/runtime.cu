@@ -1155,7 +1155,8 @@ static pic_status compact_t(pic_handle* h, int species, double* x, double* u, ui
     const int b = h->buf;
     const bool hd = h->esc == ESC_DISP;
     // arrays on this device (8-byte aligned) are written by the compaction
-    // itself, with offsets made on the device: no staging, one wait
+    // itself, with offsets made on the device: no staging, one wait.  A wrong
+    // particle count leaves the arrays as they are.
     auto in_place = [&](const void* p) { return on_device(p, h->cfg.device) && ((uintptr_t)p & 7u) == 0; };
     if (in_place(x) && in_place(u) && in_place(id) && in_place(dr)) {
         long long* off = nullptr;
@@ -1165,7 +1166,7 @@ static pic_status compact_t(pic_handle* h, int species, double* x, double* u, ui
         }
         tile_offsets_kernel<<<1, SCAN_THREADS, 0, h->stream>>>(nt, d.stay[b], d.arrv[b], d.lcount + b, d.lcap, off);
         compact_kernel<T, G><<<nt, NTHR, 0, h->stream>>>(h->tl, h->g, view_of<T>(d.arr[b]), d.stay[b], d.arrv[b], d.tcap, off, 0, 0,
-                                                       d.n, hd, x, u, id, dr);
+                                                       d.n, off + nt + 1, hd, x, u, id, dr);
         compact_loose_kernel<T, G><<<64, NTHR, 0, h->stream>>>(view_of<T>(d.larr[b]), d.lcount + b, d.lcap, 0, off + nt, d.n, hd, x, u,
                                                                id, dr);
         long long total = 0;
@@ -1233,7 +1234,7 @@ static pic_status compact_t(pic_handle* h, int species, double* x, double* u, ui
         const long long cnt = off[t1] - off[t0];
         if (cnt > 0) {
             compact_kernel<T, G><<<t1 - t0, NTHR, 0, h->stream>>>(h->tl, h->g, view_of<T>(d.arr[b]), d.stay[b], d.arrv[b],
-                                                                d.tcap, doff, t0, off[t0], cnt, hd, sx, su, sid, sdr);
+                                                                d.tcap, doff, t0, off[t0], cnt, nullptr, hd, sx, su, sid, sdr);
             e = cudaGetLastError();
             if (e == cudaSuccess) e = copy_out(off[t0], cnt);
         }
