@@ -142,7 +142,7 @@ struct pic_handle {
     void* E = nullptr;
     void* B = nullptr;
     void* J = nullptr;
-    void* Jtmp = nullptr;
+    void* Jtmp = nullptr;  // where J is not the folded current (Jcur)
     int* Jint = nullptr;  // FP32: fixed-point current the particle kernels add into
     void* Jcur = nullptr; // the folded current the field update uses (Jtmp where J holds the accumulators (FP64) or their
                           // conversion (FP32 with advection), else J)
@@ -1619,13 +1619,15 @@ pic_status pic_init(const pic_config* cfg, pic_handle** out) {
     if (DISPATCH(h, regroup_attr_t, h) != PIC_OK) return bail(PIC_ERR_CUDA);
     h->regroup_every = default_regroup_interval(h->fp64, h->tg);
     const size_t fb = (size_t)3 * g.cstride * h->esz;
+    const bool advects = (c.box == PIC_BOX_SHEAR || c.box == PIC_BOX_SHEAR_EXPAND) && AY;
+    const bool two_currents = h->fp64 || advects;  // accumulators (or their conversion) and folded current
     void** bufs[] = {&h->E, &h->B, &h->J, &h->Jtmp};
     for (void** p : bufs) {
+        if (p == &h->Jtmp && !two_currents) continue;
         if (dalloc(h, p, fb) != cudaSuccess) return bail(fail(h, PIC_ERR_OOM, "field allocation failed"));
         cudaMemsetAsync(*p, 0, fb, h->stream);
     }
-    const bool advects = (c.box == PIC_BOX_SHEAR || c.box == PIC_BOX_SHEAR_EXPAND) && AY;
-    h->Jcur = h->fp64 || advects ? h->Jtmp : h->J;
+    h->Jcur = two_currents ? h->Jtmp : h->J;
     if (advects &&
         dalloc(h, &h->adv, (size_t)2 * c.nx * sizeof(AdvCol<double>)) != cudaSuccess)
         return bail(fail(h, PIC_ERR_OOM, "allocation failed"));
