@@ -1608,6 +1608,15 @@ template <class T, int G, int NT, int STABLE, int JC> struct SmemLayout {
                                                : 32;
     static constexpr int QAB = !queue_all<G>() ? 0 : (fit >= 94 + QC ? 94 : (fit >= 64 ? fit - QC : 32));
     static_assert(QC >= 32 && (!queue_all<G>() || QAB >= 32), "a chunk's particles fit an empty queue");
+    // deal_leftovers can hand one warp a batch of both classes that share QAB
+    // entries.  With room for 64 two full batches fit.  With less, a warp
+    // leaves at most QAB - 32 entries of the two together, so all warps leave
+    // LEFT; the batches wrap around to the first warp only as its 32 and the
+    // last batch, which has at most LEFT - 32 (NW - 1) - 1 entries (a second
+    // warp would need LEFT > 32 NW).
+    static constexpr int NW = NT / 32, LEFT = NW * (QAB - 32);
+    static_assert(!queue_all<G>() || QAB >= 64 || (LEFT <= 32 * NW && 32 + LEFT - 32 * (NW - 1) - 1 <= QAB),
+                  "dealt batches of the classes that share entries do not meet");
     static constexpr int QN = QC + QAB;
     // a warp's queue: 6 QN offsets and moves, then QN cells
     static constexpr size_t QOD = (size_t)(NT / 32) * QN * 6 * sizeof(T);
