@@ -463,8 +463,6 @@ __device__ inline void tma_load_4d(void* dst, const CUtensorMap* map, int x, int
         : "memory");
 }
 
-template <class T> __device__ inline void atomic_add_shared(T* p, T v) { atomicAdd(p, v); }
-
 // Add v to the shared int32 word at shared-window address a (no return).
 __device__ inline void red_shared(uint32_t a, int v) {
     asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
@@ -472,19 +470,6 @@ __device__ inline void red_shared(uint32_t a, int v) {
 
 __device__ inline void red_shared(uint32_t a, double v) {
     asm volatile("red.shared.add.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
-}
-
-// Add v to the shared word at shared-window address a unless v is zero, as a
-// predicated reduction: no branch, so a warp whose lanes differ in which
-// contributions vanish still issues a single instruction per word.
-__device__ inline void red_shared_nz(uint32_t a, int v) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %1, 0;\n\t@p red.shared.add.s32 [%0], %1;\n\t}" ::"r"(a), "r"(v)
-                 : "memory");
-}
-__device__ inline void red_shared_nz(uint32_t a, double v) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.neu.f64 p, %1, 0d0000000000000000;\n\t@p red.shared.add.f64 [%0], %1;\n\t}" ::"r"(a),
-                 "d"(v)
-                 : "memory");
 }
 
 template <class T> __device__ inline void red_add_global(T* p, T v) { atomicAdd(p, v); }

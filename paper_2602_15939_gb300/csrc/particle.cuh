@@ -1821,7 +1821,7 @@ __device__ __forceinline__ bool tile_body(const CUtensorMap* tmE, const CUtensor
                 int cls = -1;  // deposit class: 0 core, 1 single axis, 2 full window
                 int qcell = 0;
                 int jidx = 0;
-                T o0[3], d[3];
+                T d[3];
                 if (valid) {
                     if (PREFETCH) unpack_stored<T, G>(next, LEAKY, p);
                     else load_particle<T, G>(S.in, slot_of(i), LEAKY, p);

@@ -518,7 +518,7 @@ template <class T> static JWord<T>* raw_current(pic_handle* h) {
 template <class T> static pic_status pre_particle(pic_handle* h) {
     const Grid& g = h->g;
     const long long n = 3ll * g.cstride;
-    const int blocks = (int)std::max(1ll, std::min(152ll * 8, n * (long long)sizeof(T) / (16 * NTHR * 4)));
+    const int blocks = (int)std::max(1ll, std::min(h->sms * 8ll, n * (long long)sizeof(T) / (16 * NTHR * 4)));
     pre_kernel<T><<<blocks, NTHR, 0, h->stream>>>(raw_current<T>(h), n, h->ctx, h->cc, (AdvCol<T>*)h->adv, g.nx, 0.5 * g.nx);
     h->prof.launches++;
     CK(cudaGetLastError());
@@ -554,7 +554,7 @@ template <class T, int G> static pic_status post_particles_t(pic_handle* h, cons
         StepP Pc = P;
         SpecPack<T> SPc = SP;
         void* largs[] = {(void*)&h->g, &h->tl, &Pc, &SPc, &Ep, &Bp, &Jp, &h->ctx};
-        CK(cudaLaunchKernel(h->ks.loose, dim3(152), dim3(TPB), largs, 0, h->stream));
+        CK(cudaLaunchKernel(h->ks.loose, dim3(h->sms), dim3(TPB), largs, 0, h->stream));
         h->prof.launches++;
         prof_end(h, 1);
     }
@@ -1267,7 +1267,7 @@ static pic_status sample_t(pic_handle* h, int species, uint32_t modulus, uint32_
     CK(dalloc(h, (void**)&did, sizeof(uint32_t) * m));
     CK(dalloc(h, (void**)&dcount, sizeof(unsigned long long)));
     CK(cudaMemsetAsync(dcount, 0, sizeof(unsigned long long), h->stream));
-    sample_kernel<T, G><<<std::min(h->tl.ntiles + 1, 152 * 8), NTHR, 0, h->stream>>>(
+    sample_kernel<T, G><<<std::min(h->tl.ntiles + 1, h->sms * 8), NTHR, 0, h->stream>>>(
         h->tl, view_of<T>(d.arr[b]), d.stay[b], d.arrv[b], d.tcap, view_of<T>(d.larr[b]), d.lcount + b, d.lcap, modulus,
         remainder, h->esc == ESC_DISP, max_out, dcount, dx, du, did, ddr);
     unsigned long long cnt = 0;
@@ -1309,7 +1309,7 @@ template <class T, int G> static pic_status maxwellian_t(pic_handle* h, int spec
     const int b = h->buf;
     // about four CTAs per SM in all, at most one per 256 particles of a tile
     const int per_tile = ppc * cells_per_tile;
-    const int ny = std::max(1, std::min((per_tile + NTHR - 1) / NTHR, (4 * 152 + h->tl.ntiles - 1) / h->tl.ntiles));
+    const int ny = std::max(1, std::min((per_tile + NTHR - 1) / NTHR, (4 * h->sms + h->tl.ntiles - 1) / h->tl.ntiles));
     maxwellian_kernel<T, G><<<dim3(h->tl.ntiles, ny), NTHR, 0, h->stream>>>(h->tl, h->g, ppc, theta, h->cfg.c, drift ? drift[0] : 0.0,
                                                                  drift ? drift[1] : 0.0, drift ? drift[2] : 0.0, noise, seed,
                                                                  id_base, tcap, view_of<T>(d.arr[b]), h->esc == ESC_DISP,
@@ -1655,7 +1655,7 @@ pic_status pic_init(const pic_config* cfg, pic_handle** out) {
     h->stage_elems = (size_t)3 * c.nx * c.ny * c.nz;
     if (dalloc(h, (void**)&h->stage, sizeof(double) * h->stage_elems) != cudaSuccess)
         return bail(fail(h, PIC_ERR_OOM, "staging allocation failed"));
-    h->partial_blocks = 152 * 8;
+    h->partial_blocks = h->sms * 8;
     if (dalloc(h, (void**)&h->partial, sizeof(double) * h->partial_blocks * 3 + sizeof(DiagOut)) != cudaSuccess)
         return bail(fail(h, PIC_ERR_OOM, "allocation failed"));
     if (dalloc(h, (void**)&h->err, sizeof(int)) != cudaSuccess || dalloc(h, (void**)&h->counters, 2 * sizeof(unsigned long long)) != cudaSuccess)
