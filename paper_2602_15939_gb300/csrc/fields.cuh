@@ -10,7 +10,8 @@
 // images themselves, or the shearing boxes' sweeps, which fetch the
 // (shearing-)periodic neighbours in place, and one pass that writes the new
 // fields with their guards.  Small boxes are bound by the number of dependent
-// launches (2 - 3 us each): 7 and 9 a step in place of 16 and 46.
+// launches (2 - 3 us each): 7 a step in place of 16, and of a shearing box at
+// four sweeps 9 (10 in FP32 with y active) in place of 46.
 #pragma once
 
 #include <type_traits>

@@ -1505,17 +1505,20 @@ constexpr bool has_half_shape(bool fp64, int geom) { return fp64 ? geom != G3D :
 // expanding box of 12.  Otherwise 512 threads with one.  Batched launches use
 // the same (16 3D FP32 boxes on 8^3 tiles: 1.31e10 particle-steps/s with four
 // copies against 1.24e10 with two at 256 threads).
-// FP64 (its arithmetic pipe is the bound; more registers, fewer retries of the
-// compare-and-swap adds): 256 threads, with four copies where they fit
-// (particle kernel, us: 40 x 36 x 32 on 4^3 tiles 2132 -> 1638 against 512
-// threads with one, 64^2 in 2D 246 -> 212; 64^3 on 8^3 tiles with one copy
-// 7764 -> 7114).
+// FP64 (its arithmetic pipe is the bound; more registers than the 64 of the
+// 512-thread shapes, fewer retries of the compare-and-swap adds): 256 threads,
+// with four copies where they fit (particle kernel, us: 40 x 36 x 32 on 4^3
+// tiles 2132 -> 1638 against 512 threads with one, 64^2 in 2D 246 -> 212; 64^3
+// on 8^3 tiles with one copy 7764 -> 7114).  The 3D FP64 kernels still spill:
+// tile_ctas caps them at 128 registers on 4^3 tiles (232 / 276 bytes of spill
+// stores / loads, quadratic expanding box) and 80 on 8^3 (592 / 720 bytes), for
+// two and three CTAs per SM where shared memory holds one.
 constexpr int default_tile_shape(bool fp64, int geom) {
     return has_half_shape(fp64, geom) ? HALF_SHAPE : (fp64 ? 0 : (geom == G3D ? 6 : 1));
 }
 constexpr int batch_tile_shape(bool fp64, int geom) { return default_tile_shape(fp64, geom); }
 
-// CTAs per SM the register budget is set for
+// CTAs per SM the register budget is set for (shared memory may hold fewer: 3D FP64)
 constexpr int tile_ctas(int nt, int jc) { return jc >= 4 ? (nt == 256 ? 2 : 1) : (nt == 512 ? 2 : 3); }
 
 // Dynamic shared memory: E box, B box (each 128-byte aligned, the TMA

@@ -1144,10 +1144,9 @@ template <class T, int G> static pic_status regrow_t(pic_handle* h, bool force, 
 
 // Particles of a species read back in tile order, then the loose list, into
 // the caller's buffers (host or device memory, any kind): straight into arrays
-// on this device; for other memory tiles are compacted
-// a chunk at a time into device staging buffers of at most STAGE_PARTICLES
-// particles, each chunk copied out before the next is written.
-
+// on this device; for other memory tiles are compacted a chunk at a time into
+// device staging buffers of at most STAGE_PARTICLES particles, each chunk
+// copied out before the next is written.
 template <class T, int G>
 static pic_status compact_t(pic_handle* h, int species, double* x, double* u, uint32_t* id, double* dr) {
     DevSpecies& d = h->sp[species];
