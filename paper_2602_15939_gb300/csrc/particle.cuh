@@ -334,6 +334,7 @@ template <> struct GlobalJ<float> {
         const int iv = __float_as_int(fmaf(a, b, 12582912.0f)) - 0x4B400000;
         if (iv != 0) atomicAdd(J + comp * SC + idx, iv);
     }
+    __device__ void add_w(long long word, float a, float b) const { add(0, word, a, b); }
 };
 
 template <> struct GlobalJ<double> {
@@ -344,12 +345,15 @@ template <> struct GlobalJ<double> {
         const double v = a * b;
         if (v != 0.0) red_add_global(J + comp * SC + idx, v);
     }
+    __device__ void add_w(long long word, double a, double b) const { add(0, word, a, b); }
 };
 
 // ---- gather ------------------------------------------------------------------------
 // cidx: linear index of the particle's cell in the accessor's box; o: offsets.
+// FP64 (FP32: gather_packed).
 template <class T, int G, int ORD, class F, class I>
 __device__ inline void gather(const F& fa, I cidx, const T o[3], T Ep[3], T Bp[3]) {
+    static_assert(sizeof(T) == 8, "FP32 fields are gathered by gather_packed");
     using GT = GeomT<G>;
     constexpr int NP = ORD + 1;
     T wn[3][NP], ws[3][NP];
@@ -378,12 +382,11 @@ __device__ inline void gather(const F& fa, I cidx, const T o[3], T Ep[3], T Bp[3
                     T row = wx[0] * fa.at(comp, b0 + b * fa.SY + c * fa.SZ);
 #pragma unroll
                     for (int a = 1; a < NP; ++a) row += wx[a] * fa.at(comp, b0 + a + b * fa.SY + c * fa.SZ);
-                    // FP64 (bound by its arithmetic): x, then y, then z, 39
+                    // x, then y, then z (bound by the arithmetic): 39
                     // operations a component against 45 with weight products
-                    if (sizeof(T) == 8) plane = b == 0 ? wy[0] * row : plane + wy[b] * row;
-                    else acc += (wy[b] * wz[c]) * row;
+                    plane = b == 0 ? wy[0] * row : plane + wy[b] * row;
                 }
-                if (sizeof(T) == 8) acc = c == 0 ? wz[0] * plane : acc + wz[c] * plane;
+                acc = c == 0 ? wz[0] * plane : acc + wz[c] * plane;
             }
         } else {
             constexpr int A2 = GT::AY ? 1 : 2;  // second active axis
@@ -404,14 +407,16 @@ __device__ inline void gather(const F& fa, I cidx, const T o[3], T Ep[3], T Bp[3
     Bp[0] = out[3]; Bp[1] = out[4]; Bp[2] = out[5];
 }
 
-// FP32 gather from the shared-memory boxes with packed two-wide FP32
-// arithmetic.  E_k and B_k are staggered oppositely on every axis (E_k is
+// FP32 gather with packed two-wide FP32 arithmetic.  E_k and B_k are staggered oppositely on every axis (E_k is
 // half-staggered along k only, B_k along the other two), so with the node
 // and staggered shape weights of each axis held as one pair (node, stag) --
 // or its swap (stag, node) -- every weight, row and accumulator of the pair
 // (E_k, B_k) is one packed register: each fused multiply-add does the work of
-// two, with the rounding of the scalar form.  Same weights, stencils and
-// summation order as gather().
+// two, with the rounding of the scalar form.  Tile and loose particles are
+// gathered by this one sequence of rounded operations: which particles of a
+// crowded tile go to the loose list depends on the order in which warps claim
+// slots, and the results must not.  (With gather() for the loose ones a 24^3
+// expanding box differed between two runs by 6e-8 after some 40 steps.)
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 f2swap(float2 v) { return make_float2(v.y, v.x); }
 
@@ -441,11 +446,9 @@ template <> struct Shape2<2> {
     }
 };
 
-template <int G, int ORD>
-__device__ __forceinline__ void gather_packed(const SmemFields<float, G>& fa, int cidx, const float o[3], float Ep[3],
-                                              float Bp[3]) {
+template <int G, int ORD, class FA, class I>
+__device__ __forceinline__ void gather_packed(const FA& fa, I cidx, const float o[3], float Ep[3], float Bp[3]) {
     using GT = GeomT<G>;
-    using FA = SmemFields<float, G>;
     constexpr int NP = ORD + 1;
     float2 w[3][NP];  // (node, stag) per axis
     int offn[3] = {0, 0, 0}, offs[3] = {0, 0, 0};
@@ -456,8 +459,8 @@ __device__ __forceinline__ void gather_packed(const SmemFields<float, G>& fa, in
     for (int k = 0; k < 3; ++k) {
         // E_k: staggered along k (weights .y of axis k, .x elsewhere); B_k the opposite
         float2 wk[3][NP];
-        int bE = cidx, bB = cidx;
-        constexpr int SS[3] = {1, FA::SY, FA::SZ};
+        I bE = cidx, bB = cidx;
+        const I SS[3] = {I(1), I(fa.SY), I(fa.SZ)};
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
             const bool act = ax == 0 || (ax == 1 && GT::AY) || (ax == 2 && GT::AZ);
@@ -473,22 +476,22 @@ __device__ __forceinline__ void gather_packed(const SmemFields<float, G>& fa, in
             for (int c = 0; c < NP; ++c)
 #pragma unroll
                 for (int b = 0; b < NP; ++b) {
-                    const int off = b * FA::SY + c * FA::SZ;
+                    const I off = b * I(fa.SY) + c * I(fa.SZ);
                     float2 row = f2(0.0f, 0.0f);
 #pragma unroll
                     for (int a = 0; a < NP; ++a)
-                        row = __ffma2_rn(wk[0][a], f2(fa.e[k * FA::SC + bE + off + a], fa.b[k * FA::SC + bB + off + a]), row);
+                        row = __ffma2_rn(wk[0][a], f2(fa.at(k, bE + off + a), fa.at(3 + k, bB + off + a)), row);
                     acc = __ffma2_rn(__fmul2_rn(wk[1][b], wk[2][c]), row, acc);
                 }
         } else {
             constexpr int A2 = GT::AY ? 1 : 2;
-            constexpr int S2 = A2 == 1 ? FA::SY : FA::SZ;
+            const I S2 = A2 == 1 ? I(fa.SY) : I(fa.SZ);
 #pragma unroll
             for (int b = 0; b < NP; ++b) {
                 float2 row = f2(0.0f, 0.0f);
 #pragma unroll
                 for (int a = 0; a < NP; ++a)
-                    row = __ffma2_rn(wk[0][a], f2(fa.e[k * FA::SC + bE + b * S2 + a], fa.b[k * FA::SC + bB + b * S2 + a]), row);
+                    row = __ffma2_rn(wk[0][a], f2(fa.at(k, bE + b * S2 + a), fa.at(3 + k, bB + b * S2 + a)), row);
                 acc = __ffma2_rn(wk[A2][b], row, acc);
             }
         }
@@ -999,15 +1002,15 @@ template <class T, int G, int ORD> __device__ inline int cross_mask(const T o[3]
 // particle).  The axes are taken in the cyclic order (a, a+1, a+2), with the
 // strides and component offsets picked per lane.  Same Esirkepov weights as
 // deposit(): F_bc = S0_b A_c + dS_b Q_c, symmetric in b and c.
-template <class T, int ORD, class JA>
-__device__ inline void deposit_1axis(const JA& ja, int cidx, const T o[3], const T d[3], T qs, int a) {
+template <class T, int ORD, class JA, class I>
+__device__ inline void deposit_1axis(const JA& ja, I cidx, const T o[3], const T d[3], T qs, int a) {
     constexpr int NW = ORD + 2, NC = ORD + 1;
     const int b = a == 2 ? 0 : a + 1, c = a == 0 ? 2 : a - 1;
     auto pick3 = [](const T* v, int i) -> T { return i == 0 ? v[0] : (i == 1 ? v[1] : v[2]); };
-    auto stride = [](int i) -> int { return i == 0 ? 1 : (i == 1 ? JA::SY : JA::SZ); };
+    auto stride = [&](int i) -> I { return i == 0 ? I(1) : (i == 1 ? I(ja.SY) : I(ja.SZ)); };
     const T oa = pick3(o, a), ob = pick3(o, b), oc = pick3(o, c);
     const T xa1 = oa + pick3(d, a), xb1 = ob + pick3(d, b), xc1 = oc + pick3(d, c);
-    const int sa = stride(a), sb = stride(b), sc = stride(c);
+    const I sa = stride(a), sb = stride(b), sc = stride(c);
     // axis a: the window of the full deposit; the particle moves to the next
     // node up or down, so one shape fills the lower and one the upper nodes.
     // Up or down by the arithmetic of cross_mask, not by the sign of the move:
@@ -1075,8 +1078,8 @@ __device__ inline void deposit_1axis(const JA& ja, int cidx, const T o[3], const
         Ac[m] = S0c[m] + T(0.5) * DSc[m];
         Qc[m] = T(0.5) * S0c[m] + third * DSc[m];
     }
-    const int base = cidx + wba * sa + wbb * sb + wbc * sc;
-    const int wa = base + a * JA::SC, wb = base + b * JA::SC, wc = base + c * JA::SC;
+    const I base = cidx + wba * sa + wbb * sb + wbc * sc;
+    const I wa = base + a * I(ja.SC), wb = base + b * I(ja.SC), wc = base + c * I(ja.SC);
     // The outermost loop of each component stays rolled (instruction cache, as
     // in deposit()); the values it indexes are picked by selects.
     // (windows of NC = ORD+1 nodes on b and c, NW = ORD+2 on a)
@@ -1088,11 +1091,11 @@ __device__ inline void deposit_1axis(const JA& ja, int cidx, const T o[3], const
 #pragma unroll 1
     for (int m = 0; m < NC; ++m) {
         const T s0 = pickc(S0b, m), ds = pickc(DSb, m);
-        const int mo = wa + m * sb;
+        const I mo = wa + m * sb;
 #pragma unroll
         for (int n = 0; n < NC; ++n) {
             const T f = s0 * Ac[n] + ds * Qc[n];
-            const int off = mo + n * sc;
+            const I off = mo + n * sc;
 #pragma unroll
             for (int l = 0; l < NW - 1; ++l) ja.add_w(off + l * sa, CSa[l], f);
         }
@@ -1101,11 +1104,11 @@ __device__ inline void deposit_1axis(const JA& ja, int cidx, const T o[3], const
 #pragma unroll 1
     for (int l = 0; l < NW; ++l) {
         const T s0 = pickw(S0a, l), ds = pickw(DSa, l);
-        const int lo = wb + l * sa;
+        const I lo = wb + l * sa;
 #pragma unroll
         for (int n = 0; n < NC; ++n) {
             const T f = s0 * Ac[n] + ds * Qc[n];
-            const int off = lo + n * sc;
+            const I off = lo + n * sc;
 #pragma unroll
             for (int m = 0; m < NC - 1; ++m) ja.add_w(off + m * sb, CSb[m], f);
         }
@@ -1114,11 +1117,11 @@ __device__ inline void deposit_1axis(const JA& ja, int cidx, const T o[3], const
 #pragma unroll 1
     for (int l = 0; l < NW; ++l) {
         const T s0 = pickw(S0a, l), ds = pickw(DSa, l);
-        const int lo = wc + l * sa;
+        const I lo = wc + l * sa;
 #pragma unroll
         for (int m = 0; m < NC; ++m) {
             const T f = s0 * Ab[m] + ds * Qb[m];
-            const int off = lo + m * sb;
+            const I off = lo + m * sb;
 #pragma unroll
             for (int n = 0; n < NC - 1; ++n) ja.add_w(off + n * sc, CSc[n], f);
         }
@@ -1216,7 +1219,7 @@ template <class T, int G, int ORD, int PUSH, class FA, class I>
 __device__ inline void push_particle(Particle<T>& p, const FA& fa, I fidx, const SpecStep<T>& S, const StepP& P,
                                      T d[3]) {
     T E[3], B[3];
-    if constexpr (std::is_same<FA, SmemFields<float, G>>::value) gather_packed<G, ORD>(fa, fidx, p.o, E, B);
+    if constexpr (sizeof(T) == 4) gather_packed<G, ORD>(fa, fidx, p.o, E, B);
     else gather<T, G, ORD>(fa, fidx, p.o, E, B);
     const T inv_c2 = pk<T>(P.inv_c2, P.f.inv_c2);
     if (PUSH == PUSH_KSB) {
@@ -1338,15 +1341,23 @@ __device__ inline bool move_particle(Particle<T>& p, const T d[3], const StepP& 
     return false;
 }
 
-// Push, deposit and move one particle: FA/fidx as for
-// push_particle, JA: current accumulator, jidx: the start cell's linear index
-// in its box.
+// Push, deposit and move one loose particle: FA/fidx as for push_particle, JA:
+// current accumulator, jidx: the start cell's linear index in its box.  The
+// current of the (comoving) move x^n -> x^n + d is deposited by the particle's
+// class, as tile_body does: the classes' sums round differently.
 template <class T, int G, int ORD, int PUSH, int ESC, class FA, class JA, class I>
 __device__ inline bool advance_particle(Particle<T>& p, const FA& fa, I fidx, const JA& ja, I jidx, T qs,
                                         const SpecStep<T>& S, const StepP& P, const Grid& g) {
     T d[3];
     push_particle<T, G, ORD, PUSH>(p, fa, fidx, S, P, d);
-    deposit<T, G, ORD>(ja, jidx, p.o, d, qs);  // current from the (comoving) move x^n -> x^n + d
+    const int cm = cross_mask<T, G, ORD>(p.o, d);
+    if (cm == 0) {
+        deposit_core<T, G, ORD, false>(ja, jidx, p.o, d, qs);
+    } else if (GeomT<G>::AY && GeomT<G>::AZ && (cm & (cm - 1)) == 0) {
+        if constexpr (GeomT<G>::AY && GeomT<G>::AZ) deposit_1axis<T, ORD>(ja, jidx, p.o, d, qs, cm >> 1);
+    } else {
+        deposit<T, G, ORD>(ja, jidx, p.o, d, qs);
+    }
     return move_particle<T, G, PUSH, ESC>(p, d, P, g);
 }
 
