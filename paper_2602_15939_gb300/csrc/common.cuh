@@ -86,10 +86,10 @@ template <class T> using JWord = typename JWordOf<T>::type;
 template <class T> struct ShearShift { int m, on; T w0, w1; };
 
 // Per-step, time-dependent scalars, kept in device memory so that a captured
-// CUDA graph of a step stays valid from one step to the next.  ctx_kernel
+// CUDA graph of a step stays valid from one step to the next.  ctx_update
 // fills it at the start of every step from the step counter next_step.
 struct StepCtx {
-    long long next_step;  // the step the next ctx_kernel starts (written by the host on pic_set_step)
+    long long next_step;  // the step the next ctx_update starts (written by the host on pic_set_step)
     long long step;       // n of the step in progress (fields at t^n = n)
     int dys_i[3];         // shearing shift Dy_s mod ny at t, t+1/2, t+1: integer part
     double dys_f[3];      //                                               fractional part
@@ -140,7 +140,7 @@ template <> struct CtxT<float> {
     __device__ static const ShearShift<float>& shift(const StepCtx* c, int t, int w) { return c->f_shift[t][w]; }
 };
 
-// Constants ctx_kernel needs (fixed for a handle).
+// Constants ctx_update needs (fixed for a handle).
 struct CtxConst {
     int box;        // 1 shearing, 2 expanding, 4 shearing + expanding, other: static
     int ny;
